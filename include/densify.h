@@ -344,11 +344,12 @@ DENSIFY_API void densify_reset_kernel_times(densify_ctx *ctx);
 DENSIFY_API int64_t densify_kernel_launches(densify_ctx *ctx);
 
 /* (No counterpart in the paper: a test hook for this library's error path.)
- * Makes the next batch launched on the context report what its kernels report
+ * Makes the next batch launched on the context (or the next
+ * densify_sigma_grad, whichever comes first) report what its kernels report
  * when a bounded wait on tile copies gives up: the host sets bit 0 of the
- * batch's device status word on the batch's stream, after its kernels and
- * before the status is read back (no wait on the GPU actually runs out).
- * Collecting that batch's tickets then returns DENSIFY_E_CUDA with the
+ * device status word on the work's stream, after its kernels and before the
+ * status is read back (no wait on the GPU actually runs out). Collecting that
+ * batch's tickets, or the gradient call, then returns DENSIFY_E_CUDA with the
  * bounded-wait message in densify_last_error(), and the context stays
  * unusable (every later call returns DENSIFY_E_CUDA), as after a real
  * timeout. Errors: E_INVALID (ctx NULL), E_CUDA (context already failed). */
@@ -411,7 +412,8 @@ DENSIFY_API densify_status densify_frame_noalloc(const densify_params *params, c
  * gt_depth is a device H x W float map. Synchronous: waits for in-flight
  * batches, uses arena scratch, returns when the numbers are on the host.
  * Preprocessing and contour removal are not part of it. Errors: E_INVALID,
- * E_AGAIN (scratch full), E_CUDA. */
+ * E_AGAIN (scratch full), E_CUDA (also when a kernel's bounded wait on its
+ * copies gave up; the context is unusable then, as after such a batch). */
 DENSIFY_API densify_status densify_sigma_grad(densify_ctx *ctx, const densify_frame *frame, const float *gt_depth,
                                               double *loss, double *grad, int64_t *n_pixels);
 

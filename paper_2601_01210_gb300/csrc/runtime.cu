@@ -235,7 +235,7 @@ struct densify_ctx {
     double t_us[K_COUNT] = {};
     int64_t t_n[K_COUNT] = {};
     int64_t kernel_launches = 0;   // CUDA kernels of completed batches
-    bool inject_wait_failure = false;   // densify_inject_wait_failure: armed for the next batch
+    bool inject_wait_failure = false;   // densify_inject_wait_failure: armed for the next batch or gradient
     int64_t batches = 0;                // batches launched
     int max_busy = 0;                   // most batches on the GPU at once
     bool grids_fixed = false;           // the kernel grids were settled by the first batch
@@ -1173,12 +1173,16 @@ densify_status launch_batch(densify_ctx *c, int si) {
     return DENSIFY_OK;
 }
 
+// The status word that came back with a slot's work: a kernel whose bounded wait gave up left outputs unwritten.
+densify_status check_status(densify_ctx *c, const Slot &sl) {
+    if (*sl.h_status == 0) return DENSIFY_OK;
+    c->dead = true;
+    c->err = "a kernel's bounded wait on its tile copies gave up (status " + std::to_string(*sl.h_status) + ")";
+    return DENSIFY_E_CUDA;
+}
+
 densify_status complete_slot(densify_ctx *c, Slot &sl) {
-    if (*sl.h_status != 0) {
-        c->dead = true;
-        c->err = "a kernel's bounded wait on its tile copies gave up (status " + std::to_string(*sl.h_status) + ")";
-        return DENSIFY_E_CUDA;
-    }
+    if (densify_status st = check_status(c, sl); st != DENSIFY_OK) return st;
     if (c->p.timing) {
         for (int j = 0; j < sl.seq[sl.which].ntimed; ++j) {
             const int k = sl.seq[sl.which].kord[j];
@@ -1606,9 +1610,11 @@ densify_status densify_sigma_grad(densify_ctx *c, const densify_frame *frame, co
     d.motion = nullptr;
     d.g1 = (float2 *)(base + off_g1);
     // slot 0's page-locked table (no batch is in flight): the descriptor out, then the partial sums back
-    BatchDev *hb = c->slots[0].h;
+    Slot &sl = c->slots[0];
+    BatchDev *hb = sl.h;
     std::memset(hb, 0, hdr);
     hb->n_frames = 1;
+    hb->status = sl.d_status;   // 0 (a context whose status was ever set stays failed); pooling's waits are bounded
     hb->zb_pre[1] = ceil_div((int64_t)d.zpitch * d.H, kZbWordsPerChunk);
     for (int s = 0; s < kMaxScans; ++s) hb->pt_pre[s + 1] = hb->pt_pre[s] + ceil_div(d.scans[s].count, kPtsPerChunk);
     hb->pool_pre[1] = p.num_stages == 2 ? ceil_div(d.Wc, kPoolPerChunk) * d.Hc : 0;
@@ -1625,8 +1631,9 @@ densify_status densify_sigma_grad(densify_ctx *c, const densify_frame *frame, co
         ga.s[i].inv_sc3 = (float)(1.0 / (sc * sc * sc));
         ga.s[i].inv_sp3 = (float)(1.0 / (sp * sp * sp));
     }
-    cudaStream_t s = c->slots[0].stream;
+    cudaStream_t s = sl.stream;
     BatchDev *bd = (BatchDev *)(base + off_batch);
+    int32_t *const status = hb->status;   // (hb takes the partial sums below)
     const size_t part_bytes = (size_t)grid * 6 * sizeof(float);
     std::vector<float> spill;   // (a device with so many SMs that the sums exceed the table)
     if (part_bytes > sizeof(BatchDev)) spill.resize((size_t)grid * 6);
@@ -1641,9 +1648,15 @@ densify_status densify_sigma_grad(densify_ctx *c, const densify_frame *frame, co
     if (e == cudaSuccess) e = launch_grad(bd, ga, gt, (float *)(base + off_part), grid, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(host_part, base + off_part, part_bytes, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess && c->inject_wait_failure) {   // test hook, as in launch_batch
+        e = cudaMemsetAsync(status, 1, 1, s);
+        c->inject_wait_failure = false;
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(sl.h_status, status, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     c->arena.release(r.off, total);
     if (e != cudaSuccess) return cuda_fail(c, e, "sigma gradient");
+    if (densify_status st = check_status(c, sl); st != DENSIFY_OK) return st;
     double host_out[6] = {0, 0, 0, 0, 0, 0};   // the blocks' FP32 partial sums, added on the host in FP64
     for (int b = 0; b < grid; ++b)
         for (int k = 0; k < 6; ++k) host_out[k] += (double)host_part[(size_t)b * 6 + k];

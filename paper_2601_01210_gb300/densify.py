@@ -244,7 +244,7 @@ def densify_frame_noalloc(params: densify_params, frame: densify_frame, stream: 
 
 
 def densify_inject_wait_failure(ctx) -> int:
-    """Test hook: the next batch reports a bounded wait that gave up (DENSIFY_E_CUDA)."""
+    """Test hook: the next batch or gradient reports a bounded wait that gave up (DENSIFY_E_CUDA)."""
     return lib().densify_inject_wait_failure(ctx)
 
 
