@@ -394,9 +394,26 @@ DENSIFY_API int32_t densify_describe(densify_ctx *ctx, char *buf, int32_t cap);
  * may load the library's kernel code into device memory. Later calls leave the
  * device's free memory unchanged. No cudaMalloc, cudaFree or other allocating call
  * is made. Errors: E_INVALID (bad argument or too large), E_CUDA (a launch
- * failed); the message is in densify_last_error(NULL). */
+ * failed); the message is in densify_last_error(NULL). What goes wrong on the
+ * GPU after the call returned is asked for with densify_noalloc_status(). */
 DENSIFY_API densify_status densify_frame_noalloc(const densify_params *params, const densify_frame *frame,
                                                  void *cuda_stream);
+
+/* (No counterpart in the paper.) Whether the frames that
+ * densify_frame_noalloc enqueued on the current device since the last call of
+ * this function are complete. Waits for `cuda_stream` (the stream of those
+ * calls) and returns OK, or E_CUDA when a kernel's bounded wait on its copies
+ * gave up in one of them: its outputs are then incomplete, and the message is
+ * in densify_last_error(NULL). The record is cleared, so later frames start
+ * anew. Makes no device allocation; not for a stream that is being captured.
+ * Errors: E_CUDA (also when the stream's work failed). */
+DENSIFY_API densify_status densify_noalloc_status(void *cuda_stream);
+
+/* (No counterpart in the paper: a test hook for this library's error path.)
+ * The calling thread's next densify_frame_noalloc reports what its kernels
+ * report when a bounded wait gives up: the host sets the status bit on its
+ * stream, after the kernels (no wait on the GPU actually runs out). */
+DENSIFY_API densify_status densify_inject_noalloc_wait_failure(void);
 
 /* Gradient of the depth error with respect to the filter's sigmas (Sec. 4:
  * when dense ground truth exists, the Gaussian variances can be optimised by

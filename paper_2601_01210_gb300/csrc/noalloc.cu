@@ -10,8 +10,11 @@
 // first call made with that device current) the entry point asks the runtime
 // for the array's device address with cudaGetSymbolAddress and passes that
 // pointer to the kernels. Everything the kernels read is rewritten or cleared
-// on every call: the descriptor and status by a one-block init kernel, the
-// z-buffer by the clear kernel, the other maps before they are read.
+// on every call: the descriptor by a one-block init kernel, the z-buffer by
+// the clear kernel, the other maps before they are read. The status word, which
+// the kernels only set (a bounded wait on tile copies that gave up, the frame's
+// outputs then incomplete), keeps its bits until densify_noalloc_status reads
+// them, so that a caller with several frames enqueued misses none.
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -41,6 +44,11 @@ struct DeviceSetup {
 std::mutex g_setup_mu;
 DeviceSetup g_setup[kMaxDevices];
 
+// The scratch begins with the batch descriptor of one frame, then the status word.
+constexpr size_t kOffStatus = (offsetof(BatchDev, f) + sizeof(FrameDev) + 255) & ~size_t(255);
+
+thread_local bool g_inject_wait_failure = false;   // densify_inject_noalloc_wait_failure: armed for the thread's next call
+
 // Frame descriptor passed by value as raw words (its tensor-map members are
 // 64-byte aligned, which kernel parameters do not guarantee).
 struct FrameWords {
@@ -59,7 +67,6 @@ __global__ void noalloc_init_kernel(BatchDev *b, FrameWords f, Prefix p, int32_t
     if (threadIdx.x == 0) {
         b->n_frames = 1;
         b->status = status;
-        *status = 0;
         b->zb_pre[0] = 0;
         b->zb_pre[1] = p.zb;
         b->pt_pre[0] = 0;
@@ -133,11 +140,7 @@ extern "C" DENSIFY_API densify_status densify_frame_noalloc(const densify_params
     const int zpitch = (W + 3) & ~3, cpitch = (Wc + 3) & ~3;
     const int64_t npx = (int64_t)W * H;
     const int n_bp = cdiv(npx, kBpChunk);
-    size_t o = 0;
-    const size_t off_batch = o;
-    o += up256(offsetof(BatchDev, f) + sizeof(FrameDev));
-    const size_t off_status = o;
-    o += 256;
+    size_t o = kOffStatus + 256;
     const size_t off_zbuf = o;
     o += up256((size_t)zpitch * H * 4);
     size_t off_cg = 0, off_cs = 0, off_s1 = 0;
@@ -282,8 +285,8 @@ extern "C" DENSIFY_API densify_status densify_frame_noalloc(const densify_params
         fill_stage_args(sa[1], params->stage[1], params->pool, params->stage2_input);
     }
 
-    BatchDev *b = reinterpret_cast<BatchDev *>(base + off_batch);
-    int32_t *status = reinterpret_cast<int32_t *>(base + off_status);
+    BatchDev *b = reinterpret_cast<BatchDev *>(base);
+    int32_t *status = reinterpret_cast<int32_t *>(base + kOffStatus);
     const int sms = setup.sms;
     noalloc_init_kernel<<<1, 128, 0, s>>>(b, fw, pre, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(DENSIFY_E_CUDA, cudaGetErrorString(e));
@@ -322,6 +325,44 @@ extern "C" DENSIFY_API densify_status densify_frame_noalloc(const densify_params
     if (f->out_zbuf)
         NA_TRY(cudaMemcpy2DAsync(f->out_zbuf, (size_t)W * 4, d.zbuf, (size_t)zpitch * 4, (size_t)W * 4, (size_t)H,
                                  cudaMemcpyDeviceToDevice, s));
+    if (g_inject_wait_failure) {   // test hook: the bit a kernel sets when a bounded wait gives up
+        g_inject_wait_failure = false;
+        NA_TRY(cudaMemsetAsync(status, 1, 1, s));
+    }
 #undef NA_TRY
+    return DENSIFY_OK;
+}
+
+extern "C" DENSIFY_API densify_status densify_noalloc_status(void *cuda_stream) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return fail(DENSIFY_E_CUDA, std::string("cudaGetDevice: ") + cudaGetErrorString(e));
+    if (dev < 0 || dev >= kMaxDevices) return fail(DENSIFY_E_INVALID, "device index too large");
+    unsigned char *base = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_setup_mu);
+        base = g_setup[dev].scratch;
+    }
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    int32_t status = 0;
+    if (base) {   // some call ran on this device
+        e = cudaMemcpyAsync(&status, base + kOffStatus, sizeof(status), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess && status) {
+            e = cudaMemsetAsync(base + kOffStatus, 0, sizeof(status), s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        }
+    } else {
+        e = cudaStreamSynchronize(s);
+    }
+    if (e != cudaSuccess) return fail(DENSIFY_E_CUDA, std::string("status: ") + cudaGetErrorString(e));
+    if (status)
+        return fail(DENSIFY_E_CUDA, "a kernel's bounded wait on its tile copies gave up (status " +
+                                        std::to_string(status) + "): outputs are incomplete");
+    return DENSIFY_OK;
+}
+
+extern "C" DENSIFY_API densify_status densify_inject_noalloc_wait_failure(void) {
+    g_inject_wait_failure = true;
     return DENSIFY_OK;
 }

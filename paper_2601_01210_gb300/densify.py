@@ -123,7 +123,9 @@ _SIGS = {
     "densify_sigma_grad": ([C.c_void_p, C.POINTER(densify_frame), C.c_void_p, C.POINTER(C.c_double),
                             C.POINTER(C.c_double), C.POINTER(C.c_int64)], C.c_int),
     "densify_frame_noalloc": ([C.POINTER(densify_params), C.POINTER(densify_frame), C.c_void_p], C.c_int),
+    "densify_noalloc_status": ([C.c_void_p], C.c_int),
     "densify_inject_wait_failure": ([C.c_void_p], C.c_int),
+    "densify_inject_noalloc_wait_failure": ([], C.c_int),
 }
 EXPORTED = tuple(_SIGS)
 
@@ -243,9 +245,20 @@ def densify_frame_noalloc(params: densify_params, frame: densify_frame, stream: 
     return lib().densify_frame_noalloc(C.byref(params), C.byref(frame), C.c_void_p(stream or 0))
 
 
+def densify_noalloc_status(stream: int | None = None) -> int:
+    """Waits for ``stream``; DENSIFY_E_CUDA when a frame that densify_frame_noalloc enqueued since the
+    last call is incomplete (densify_last_error(None) says why)."""
+    return lib().densify_noalloc_status(C.c_void_p(stream or 0))
+
+
 def densify_inject_wait_failure(ctx) -> int:
     """Test hook: the next batch or gradient reports a bounded wait that gave up (DENSIFY_E_CUDA)."""
     return lib().densify_inject_wait_failure(ctx)
+
+
+def densify_inject_noalloc_wait_failure() -> int:
+    """Test hook: this thread's next densify_frame_noalloc reports a bounded wait that gave up."""
+    return lib().densify_inject_noalloc_wait_failure()
 
 
 # ---------------------------------------------------------------------------
