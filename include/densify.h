@@ -390,8 +390,9 @@ DENSIFY_API int32_t densify_describe(densify_ctx *ctx, char *buf, int32_t cap);
  * The first call on a device looks up the array's device address and the SM
  * count (once per device, with that device current); make that first call
  * before any stream capture, and before the device-memory footprint is
- * frozen: like the first launch of any kernel under lazy module loading, it
- * may load the library's kernel code into device memory. Later calls leave the
+ * frozen: it loads the code of every kernel that some later call may take
+ * (which depends on the parameters and on the frame's alignment) into device
+ * memory. Later calls leave the
  * device's free memory unchanged. No cudaMalloc, cudaFree or other allocating call
  * is made. Errors: E_INVALID (bad argument or too large), E_CUDA (a launch
  * failed); the message is in densify_last_error(NULL). What goes wrong on the

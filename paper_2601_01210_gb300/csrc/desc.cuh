@@ -220,6 +220,9 @@ cudaError_t launch_bp_write(const BatchDev *b, int grid, cudaStream_t s);
 cudaError_t launch_bp_rows(const BatchDev *b, int radius, int grid, cudaStream_t s);
 int occupancy_points(KernelId k);
 int occupancy_pool_bp(KernelId k);
+// load_*: the kernels' code onto the device now (it is otherwise loaded at a kernel's first launch)
+cudaError_t load_points();
+cudaError_t load_pool_bp();
 
 // Joint bilateral filter, one entry per stage kind:
 //   single: full resolution, z-buffer input (radii 1-7)
@@ -232,6 +235,9 @@ cudaError_t launch_jbf_up(int radius, const BatchDev *b, const StageArgs &a, int
 int occupancy_jbf_single(int radius);
 int occupancy_jbf_coarse(int radius);
 int occupancy_jbf_up(int radius);
+cudaError_t load_jbf_single(int radius);
+cudaError_t load_jbf_coarse(int radius);
+cudaError_t load_jbf_up(int radius);
 int kp_jbf_single(int radius);
 int kp_jbf_coarse(int radius);
 int kp_jbf_up(int radius);

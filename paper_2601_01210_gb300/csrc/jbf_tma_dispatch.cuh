@@ -48,12 +48,18 @@ int occ() {
     return n > 0 ? n : 1;
 }
 
+template <int SRC, int R, int KP, int FORM, int NW>
+cudaError_t load() {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, jbf_tma_kernel<SRC, R, KP, FORM, NW>);
+}
+
 }  // namespace tma_detail
 }  // namespace dz
 
-// Defines the five lookups of one translation unit's instantiation list
+// Defines the six lookups of one translation unit's instantiation list
 // CASES(X), X(source, radius, rows per thread, form, warps), under the names
-// PREFIX_variants / _info / _prepare / _launch / _occupancy.
+// PREFIX_variants / _info / _prepare / _load / _launch / _occupancy.
 #define DZ_TMA_LOOKUPS(CASES, PREFIX)                                                                              \
     int PREFIX##_variants(int src, int r, int form, TmaVariant *out, int cap) {                                   \
         int n = 0;                                                                                                 \
@@ -66,6 +72,10 @@ int occ() {
     }                                                                                                              \
     cudaError_t PREFIX##_prepare(int src, int r, TmaVariant v, int form) {                                        \
         CASES(DZ_TMA_X_PREPARE)                                                                                    \
+        return cudaErrorInvalidValue;                                                                              \
+    }                                                                                                              \
+    cudaError_t PREFIX##_load(int src, int r, TmaVariant v, int form) {                                           \
+        CASES(DZ_TMA_X_LOAD)                                                                                       \
         return cudaErrorInvalidValue;                                                                              \
     }                                                                                                              \
     cudaError_t PREFIX##_launch(int src, int r, TmaVariant v, int form, const BatchDev *b, const StageArgs &a,    \
@@ -85,6 +95,8 @@ int occ() {
     if (DZ_TMA_MATCH(S, RR, K, F, NW)) { tma_detail::fill_info<S, RR, K, F, NW>(out); return true; }
 #define DZ_TMA_X_PREPARE(S, RR, K, F, NW) \
     if (DZ_TMA_MATCH(S, RR, K, F, NW)) return tma_detail::prep<S, RR, K, F, NW>();
+#define DZ_TMA_X_LOAD(S, RR, K, F, NW) \
+    if (DZ_TMA_MATCH(S, RR, K, F, NW)) return tma_detail::load<S, RR, K, F, NW>();
 #define DZ_TMA_X_LAUNCH(S, RR, K, F, NW) \
     if (DZ_TMA_MATCH(S, RR, K, F, NW)) return tma_detail::go<S, RR, K, F, NW>(b, a, grid, s);
 #define DZ_TMA_X_OCC(S, RR, K, F, NW) \

@@ -264,6 +264,18 @@ cudaError_t jbf_block_prepare(int r, TmaVariant v) {
     return cudaErrorInvalidValue;
 }
 
+cudaError_t jbf_block_load(int r, TmaVariant v) {
+    cudaFuncAttributes at;
+#define DZ_X(R, NW)                                                                       \
+    if (r == R && v.nw == NW) {                                                           \
+        const cudaError_t e = cudaFuncGetAttributes(&at, jbf_block_kernel<R, NW, false>); \
+        return e != cudaSuccess ? e : cudaFuncGetAttributes(&at, jbf_block_kernel<R, NW, true>); \
+    }
+    DZ_BLOCK_CASES(DZ_X)
+#undef DZ_X
+    return cudaErrorInvalidValue;
+}
+
 cudaError_t jbf_block_launch(int r, TmaVariant v, bool points, const BatchDev *b, const StageArgs &a, int grid, cudaStream_t s) {
 #define DZ_X(R, NW)                                                                                         \
     if (r == R && v.nw == NW) {                                                                             \

@@ -20,6 +20,12 @@ int occ() {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, jbf_kernel<JBF_COARSE, R, Kp<R>::value>, 256, 0);
     return n > 0 ? n : 1;
 }
+
+template <int R>
+cudaError_t load() {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, jbf_kernel<JBF_COARSE, R, Kp<R>::value>);
+}
 }  // namespace
 
 cudaError_t launch_jbf_coarse(int radius, const BatchDev *b, const StageArgs &a, int grid, cudaStream_t s) {
@@ -45,6 +51,19 @@ int occupancy_jbf_coarse(int radius) {
     case 6: return occ<6>();
     case 7: return occ<7>();
     default: return 1;
+    }
+}
+
+cudaError_t load_jbf_coarse(int radius) {
+    switch (radius) {
+    case 1: return load<1>();
+    case 2: return load<2>();
+    case 3: return load<3>();
+    case 4: return load<4>();
+    case 5: return load<5>();
+    case 6: return load<6>();
+    case 7: return load<7>();
+    default: return cudaErrorInvalidValue;
     }
 }
 

@@ -140,6 +140,14 @@ cudaError_t jbf_list_prepare(int r, TmaVariant v) {
     return cudaErrorInvalidValue;
 }
 
+cudaError_t jbf_list_load(int r, TmaVariant v) {
+    cudaFuncAttributes at;
+#define DZ_X(R, BL) if (r == R && v.kp == BL) return cudaFuncGetAttributes(&at, jbf_list_kernel<R, BL>);
+    DZ_LIST_CASES(DZ_X)
+#undef DZ_X
+    return cudaErrorInvalidValue;
+}
+
 cudaError_t jbf_list_launch(int r, TmaVariant v, const BatchDev *b, const StageArgs &a, int grid, cudaStream_t s) {
 #define DZ_X(R, BL)                                                                    \
     if (r == R && v.kp == BL) {                                                        \

@@ -56,6 +56,19 @@ cudaError_t jbf_tma_prepare(int src, int r, TmaVariant v, int form) {
                                     : base_prepare(src, r, v, form);
 }
 
+cudaError_t jbf_tma_load(int src, int r, TmaVariant v, int form) {
+    if (form == TMA_FORM_LIST) return jbf_list_load(r, v);
+    if (form == TMA_FORM_BLOCK) return jbf_block_load(r, v);
+    return form == TMA_FORM_SPARSE ? jbf_tma_sp_load(src, r, v, form)
+           : form >= TMA_FORM_EXP   ? jbf_tma_exp_load(src, r, v, form)
+                                    : base_load(src, r, v, form);
+}
+
+cudaError_t load_tile_mark() {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, tile_mark_kernel<SRC_ZBUF>);
+}
+
 cudaError_t launch_jbf_tma(int src, int r, TmaVariant v, int form, const BatchDev *b, const StageArgs &a, int grid,
                            cudaStream_t s) {
     if (form == TMA_FORM_LIST) return jbf_list_launch(r, v, b, a, grid, s);

@@ -20,6 +20,12 @@ int occ() {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, jbf_kernel<JBF_UP, R, Kp<R>::value>, 256, 0);
     return n > 0 ? n : 1;
 }
+
+template <int R>
+cudaError_t load() {
+    cudaFuncAttributes at;
+    return cudaFuncGetAttributes(&at, jbf_kernel<JBF_UP, R, Kp<R>::value>);
+}
 }  // namespace
 
 cudaError_t launch_jbf_up(int radius, const BatchDev *b, const StageArgs &a, int grid, cudaStream_t s) {
@@ -37,6 +43,15 @@ int occupancy_jbf_up(int radius) {
     case 2: return occ<2>();
     case 3: return occ<3>();
     default: return 1;
+    }
+}
+
+cudaError_t load_jbf_up(int radius) {
+    switch (radius) {
+    case 1: return load<1>();
+    case 2: return load<2>();
+    case 3: return load<3>();
+    default: return cudaErrorInvalidValue;
     }
 }
 

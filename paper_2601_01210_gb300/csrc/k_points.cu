@@ -227,6 +227,12 @@ cudaError_t launch_project(const BatchDev *b, int grid, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+cudaError_t load_points() {
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, prep_kernel);
+    return e != cudaSuccess ? e : cudaFuncGetAttributes(&at, project_kernel);
+}
+
 int occupancy_points(KernelId k) {
     int n = 0;
     if (k == K_PREP) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, prep_kernel, kThreads, 0);

@@ -720,6 +720,16 @@ cudaError_t launch_bp_write(const BatchDev *b, int grid, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+cudaError_t load_pool_bp() {
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, pool_kernel);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, bp_rows_kernel);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, bp_count_kernel);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, bp_scan_kernel);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, bp_write_kernel);
+    return e;
+}
+
 int occupancy_pool_bp(KernelId k) {
     int n = 0;
     if (k == K_POOL) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pool_kernel, kThreads, 0);

@@ -98,6 +98,28 @@ __global__ void noalloc_init_kernel(BatchDev *b, FrameWords f, Prefix p, int32_t
 size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 int cdiv(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
+// Loads every kernel that some frame or parameters may take, whichever route they then go: code that is
+// loaded lazily, at a kernel's first launch, takes device memory.
+cudaError_t load_kernels() {
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, noalloc_init_kernel);
+    if (e == cudaSuccess) e = load_points();
+    if (e == cudaSuccess) e = load_pool_bp();
+    if (e == cudaSuccess) e = load_tile_mark();
+    for (int r = 1; r <= kMaxR && e == cudaSuccess; ++r) {
+        e = load_jbf_single(r);
+        if (e == cudaSuccess) e = load_jbf_coarse(r);
+        if (e == cudaSuccess && r <= 3) e = load_jbf_up(r);
+        // FP32 contexts' default kernels: the first variant of a form
+        for (int src : {TMA_SRC_UP, TMA_SRC_ZBUF, TMA_SRC_COARSE})
+            for (int form = 0; form <= TMA_FORM_LIST && e == cudaSuccess; ++form) {
+                TmaVariant v;
+                if (form != TMA_FORM_FP16 && jbf_tma_variants(src, r, form, &v, 1) == 1) e = jbf_tma_load(src, r, v, form);
+            }
+    }
+    return e;
+}
+
 densify_status fail(densify_status s, const std::string &m) {
     set_thread_error(m);
     return s;
@@ -194,6 +216,8 @@ extern "C" DENSIFY_API densify_status densify_frame_noalloc(const densify_params
                 return fail(DENSIFY_E_CUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
             if ((e = cudaDeviceGetAttribute(&S.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
                 return fail(DENSIFY_E_CUDA, std::string("device attribute: ") + cudaGetErrorString(e));
+            if ((e = load_kernels()) != cudaSuccess)
+                return fail(DENSIFY_E_CUDA, std::string("kernel load: ") + cudaGetErrorString(e));
             S.scratch = static_cast<unsigned char *>(p);
             S.ready = true;
         }

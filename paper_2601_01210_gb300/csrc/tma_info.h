@@ -46,17 +46,20 @@ constexpr double kExpRange = 100.0;
 int jbf_tma_variants(int src, int r, int form, TmaVariant *out, int cap);
 bool jbf_tma_info(int src, int r, TmaVariant v, int form, TmaKernelInfo *out);
 cudaError_t jbf_tma_prepare(int src, int r, TmaVariant v, int form);
+cudaError_t jbf_tma_load(int src, int r, TmaVariant v, int form);   // its code onto the device now
 cudaError_t launch_jbf_tma(int src, int r, TmaVariant v, int form, const BatchDev *b, const StageArgs &a, int grid,
                            cudaStream_t s);
 int occupancy_jbf_tma(int src, int r, TmaVariant v, int form);
 // Flag the tiles of the stage's grid (tw x th) that some observation within radius r
 // reaches (the flags were zeroed by the batch's first kernel).
 cudaError_t launch_tile_mark(int src, const BatchDev *b, int stage, int th, int r, int grid, cudaStream_t s);
+cudaError_t load_tile_mark();   // (a single stage's, on the z-buffer)
 
 // the expanded form's instantiations (k_jbf_tma_exp.cu)
 int jbf_tma_exp_variants(int src, int r, int form, TmaVariant *out, int cap);
 bool jbf_tma_exp_info(int src, int r, TmaVariant v, int form, TmaKernelInfo *out);
 cudaError_t jbf_tma_exp_prepare(int src, int r, TmaVariant v, int form);
+cudaError_t jbf_tma_exp_load(int src, int r, TmaVariant v, int form);
 cudaError_t jbf_tma_exp_launch(int src, int r, TmaVariant v, int form, const BatchDev *b, const StageArgs &a,
                                int grid, cudaStream_t s);
 int jbf_tma_exp_occupancy(int src, int r, TmaVariant v, int form);
@@ -65,6 +68,7 @@ int jbf_tma_exp_occupancy(int src, int r, TmaVariant v, int form);
 int jbf_tma_sp_variants(int src, int r, int form, TmaVariant *out, int cap);
 bool jbf_tma_sp_info(int src, int r, TmaVariant v, int form, TmaKernelInfo *out);
 cudaError_t jbf_tma_sp_prepare(int src, int r, TmaVariant v, int form);
+cudaError_t jbf_tma_sp_load(int src, int r, TmaVariant v, int form);
 cudaError_t jbf_tma_sp_launch(int src, int r, TmaVariant v, int form, const BatchDev *b, const StageArgs &a,
                               int grid, cudaStream_t s);
 int jbf_tma_sp_occupancy(int src, int r, TmaVariant v, int form);
@@ -73,6 +77,7 @@ int jbf_tma_sp_occupancy(int src, int r, TmaVariant v, int form);
 int jbf_block_variants(int r, TmaVariant *out, int cap);
 bool jbf_block_info(int r, TmaVariant v, TmaKernelInfo *out);
 cudaError_t jbf_block_prepare(int r, TmaVariant v);
+cudaError_t jbf_block_load(int r, TmaVariant v);
 // points: the kernel writes the frames' points as well (FrameDev::row_pre, seg_pre)
 cudaError_t jbf_block_launch(int r, TmaVariant v, bool points, const BatchDev *b, const StageArgs &a, int grid, cudaStream_t s);
 int jbf_block_occupancy(int r, TmaVariant v);
@@ -81,6 +86,7 @@ int jbf_block_occupancy(int r, TmaVariant v);
 int jbf_list_variants(int r, TmaVariant *out, int cap);
 bool jbf_list_info(int r, TmaVariant v, TmaKernelInfo *out);
 cudaError_t jbf_list_prepare(int r, TmaVariant v);
+cudaError_t jbf_list_load(int r, TmaVariant v);
 cudaError_t jbf_list_launch(int r, TmaVariant v, const BatchDev *b, const StageArgs &a, int grid, cudaStream_t s);
 int jbf_list_occupancy(int r, TmaVariant v);
 
