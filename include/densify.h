@@ -360,7 +360,8 @@ DENSIFY_API densify_status densify_inject_wait_failure(densify_ctx *ctx);
  * chosen kernel (TMA-staged or plain, rows per thread, tile, grid) and, after
  * autotuning, every candidate's measured time; then the number of batches
  * launched and the most batches in flight at once (launched, not yet
- * complete). Writes at most cap bytes
+ * complete), and the number of CUDA graphs captured (all of them by the first
+ * batch). Writes at most cap bytes
  * (NUL-terminated); returns the length of the full text. */
 DENSIFY_API int32_t densify_describe(densify_ctx *ctx, char *buf, int32_t cap);
 

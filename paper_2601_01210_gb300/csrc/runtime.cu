@@ -8,8 +8,9 @@
 // * Batching: admitted frames queue on the host. A batch slot takes up to
 //   max_batch of them, writes their descriptors into its device table and
 //   runs the fixed kernel sequence (prep, project, [pool, coarse filter],
-//   filter, compaction count, compaction write) on the context stream,
-//   replayed from a CUDA graph captured the first time the slot is used.
+//   filter, compaction count, compaction write, or the points from the second
+//   filter) on the context stream, replayed from a CUDA graph that the
+//   context's first batch captured.
 //   Frames that arrive while every slot is busy go out together as soon as a
 //   slot frees (continuous batching).
 // * Completion: each slot records an event; densify_poll() queries events
@@ -239,6 +240,8 @@ struct densify_ctx {
     int64_t batches = 0;                // batches launched
     int max_busy = 0;                   // most batches on the GPU at once
     bool grids_fixed = false;           // the kernel grids were settled by the first batch
+    bool sequences_ready = false;       // the graphs (or kernels) of both sequences are there
+    int graphs = 0;                     // graphs captured
 };
 
 namespace {
@@ -1019,6 +1022,7 @@ densify_status capture_slot(densify_ctx *c, Slot &sl, int which) {
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_fail(c, e, "graph instantiate");
     CU(cudaGraphUpload(sl.seq[which].exec, sl.stream), "graph upload");
+    ++c->graphs;
     return DENSIFY_OK;
 }
 
@@ -1027,8 +1031,11 @@ densify_status capture_slot(densify_ctx *c, Slot &sl, int which) {
 // (one such frame keeps the eight kernels that the launch counter is tested on; its kernels last a few
 // microseconds each either way).
 constexpr int64_t kFusedPointsPx = 1 << 19;
+bool may_write_points(const densify_ctx *c) {   // some batch of this context
+    return fused_points_apply(c->p) && c->sel[1].tma && c->sel[1].form == TMA_FORM_BLOCK;
+}
 bool batch_writes_points(const densify_ctx *c, const std::vector<uint64_t> &tk) {
-    if (!fused_points_apply(c->p) || c->sel[1].form != TMA_FORM_BLOCK || !c->sel[1].tma) return false;
+    if (!may_write_points(c)) return false;
     int64_t px = 0;
     for (uint64_t t : tk) {
         const FrameRec &r = c->frames.at(t);
@@ -1036,6 +1043,27 @@ bool batch_writes_points(const densify_ctx *c, const std::vector<uint64_t> &tk) 
         px += (int64_t)r.fr.K.width * r.fr.K.height;
     }
     return px > kFusedPointsPx;
+}
+
+// The first batch captures, instantiates and uploads the graphs of both kernel sequences for every slot
+// (they are fixed once the filter kernels are chosen), so that no later batch pays for a capture, whatever
+// its size; without graphs it loads the second sequence's kernels. (Captured when a batch first took it,
+// the second sequence cost that batch 60 to 90 us in mid-traffic with two slots.)
+densify_status prepare_sequences(densify_ctx *c) {
+    if (c->sequences_ready) return DENSIFY_OK;
+    const int n = may_write_points(c) ? 2 : 1;
+    if (c->p.use_graphs) {
+        for (int which = 0; which < n; ++which)
+            for (auto &sl : c->slots) {
+                densify_status st = capture_slot(c, sl, which);
+                if (st != DENSIFY_OK) return st;
+            }
+    } else if (n == 2) {
+        CU(jbf_block_load(c->sel[1].radius, TmaVariant{c->sel[1].kp, c->sel[1].nw}), "kernel load");
+        CU(load_pool_bp(), "kernel load");
+    }
+    c->sequences_ready = true;
+    return DENSIFY_OK;
 }
 
 densify_status launch_batch(densify_ctx *c, int si) {
@@ -1098,14 +1126,8 @@ densify_status launch_batch(densify_ctx *c, int si) {
                              sl.stream),
            "rgb staging");
     }
+    if (densify_status st = prepare_sequences(c); st != DENSIFY_OK) return st;
     if (c->p.use_graphs) {
-        // the first batch of a sequence captures, instantiates and uploads every slot's graph of it (the
-        // kernel sequence is fixed once the filter kernels are chosen), so no later one pays for a capture
-        for (auto &other : c->slots) {
-            if (other.seq[which].exec) continue;
-            densify_status st = capture_slot(c, other, which);
-            if (st != DENSIFY_OK) return st;
-        }
         CU(cudaGraphLaunch(sl.seq[which].exec, sl.stream), "graph launch");
     } else {
         densify_status st = issue_kernels(c, sl, which, sl.stream, c->p.timing != 0);
@@ -1702,7 +1724,7 @@ int32_t densify_describe(densify_ctx *c, char *buf, int32_t cap) {
         out += "]}";
     }
     out += "], \"batches\": {\"launched\": " + std::to_string(c->batches) +
-           ", \"max_in_flight\": " + std::to_string(c->max_busy) + "}}";
+           ", \"max_in_flight\": " + std::to_string(c->max_busy) + "}, \"graphs\": " + std::to_string(c->graphs) + "}";
     if (buf && cap > 0) {
         const size_t n = std::min<size_t>(out.size(), (size_t)cap - 1);
         std::memcpy(buf, out.data(), n);
