@@ -54,6 +54,12 @@ def tap_form(chosen, default):
     return chosen.get("form", default) if loop == "gather" else loop
 
 
+def stage2_roof_us(work, points, taps_per_s, hbm):
+    """Roofline time of the second filter: its taps, or, where it writes the points too, its bytes."""
+    us = work["taps2"] / taps_per_s * 1e6
+    return max(us, work["stage2_points"] / hbm * 1e6) if points else us
+
+
 def parse():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -309,10 +315,10 @@ def config_measure(name, cfg, views, a, dev, stream, flush_buf, tap_peak, hbm):
     forms = [tap_form(st["chosen"], "fp32") for st in choice["stages"]]
     roof = {k: work[k] / hbm * 1e6 for k in ("prep_compose_clear", "motion_mask", "motion_dilate", "motion_erode",
                                               "project_zbuf", "occlusion", "pool3", "tile_mark1", "contour",
-                                              "bp_count", "bp_write") if k in work}
+                                              "bp_count", "bp_write", "bp_rows") if k in work}
     roof["jbf_stage1"] = work["taps1"] / tap_peak(forms[0])[0] * 1e6
     if ns == 2:
-        roof["jbf_stage2"] = work["taps2"] / tap_peak(forms[1])[0] * 1e6
+        roof["jbf_stage2"] = stage2_roof_us(work, "bp_rows" in ktable, tap_peak(forms[1])[0], hbm)
     kroof = {k: {"roof_us": round(r, 2), "measured_us": ktable[k]["avg_us"],
                  "frac": round(r / ktable[k]["avg_us"], 3) if ktable[k]["avg_us"] else None}
              for k, r in roof.items() if k in ktable}
@@ -632,6 +638,11 @@ def step_work(b, view, pool=3, single_radius=None, prepost=None):
         "tile_mark1": 4 * Wc * Hc,                            # one observation word per pooled pixel
         "bp_count": W * H,                                    # validity bytes
         "bp_write": 8 * W * H + 16 * nout,                    # validity, depth, colour in; points out
+        # where the second filter writes the points (bp_rows in the kernel table): a validity bit a pooled
+        # pixel in, a word a row and 96-column segment out; colour and first-stage result in, depth,
+        # validity and points out
+        "bp_rows": Wc * Hc // 8 + 4 * H * (1 + -(-W // 96)),
+        "stage2_points": 8 * W * H + 8 * Wc * Hc + 16 * nout,
         "taps1": valid_taps_stage1(cnt_pos),
         "taps2": valid_taps_stage2(b.coarse_valid.cpu().numpy(), W, H),
         **extra,
@@ -907,9 +918,9 @@ def ours_arm(a, rank, world, local_rank):
     hbm = peaks.get("hbm_gbs", 6758.5) * 1e9
     alu = lambda form: tap_peak(form)[0]   # taps per second
     roof_us = {k: work[k] / hbm * 1e6 for k in ("prep_compose_clear", "project_zbuf", "pool3", "tile_mark1",
-                                                "bp_count", "bp_write")}
+                                                "bp_count", "bp_write", "bp_rows")}
     roof_us["jbf_stage1"] = work["taps1"] / alu(form1) * 1e6
-    roof_us["jbf_stage2"] = work["taps2"] / alu(form2) * 1e6
+    roof_us["jbf_stage2"] = stage2_roof_us(work, "bp_rows" in ktable, alu(form2), hbm)
     kroof = {k: {"roof_us": round(r, 2), "measured_us": ktable[k]["avg_us"],
                  "frac": round(r / ktable[k]["avg_us"], 3) if ktable.get(k, {}).get("avg_us") else None}
              for k, r in roof_us.items() if k in ktable}

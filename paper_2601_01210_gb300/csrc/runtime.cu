@@ -46,7 +46,7 @@ namespace {
 const char *const kKernelNames[K_COUNT] = {"prep_compose_clear", "motion_mask", "motion_dilate", "motion_erode",
                                            "project_zbuf",       "occlusion",   "pool3",         "jbf_stage1",
                                            "jbf_stage2",         "contour",     "bp_count",      "bp_write",
-                                           "tile_mark1"};
+                                           "tile_mark1",         "bp_rows"};
 
 constexpr uint64_t kAlign = 256;
 uint64_t align_up(uint64_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
@@ -962,7 +962,7 @@ densify_status issue_kernels(densify_ctx *c, Slot &sl, int which, cudaStream_t s
         CU(mark(K_JBF1), "event");
         if (points) {
             CU(launch_bp_rows(b, c->sel[1].radius, c->sms * 4, s), "row prefix launch");
-            CU(mark(K_BP_COUNT), "event");
+            CU(mark(K_BP_ROWS), "event");
         }
         CU(start_last(), "event");
         CU(launch_filter_kernel(c, 1, b, s, points), "stage-2 filter launch");
