@@ -42,7 +42,7 @@ UNIT = "frames/s"
 # issue slots of one filter tap in each arithmetic form: the last-resort peak model, used only when
 # neither the committed nor a live measurement of the instruction rates is available
 # (block: its FMA pipe's 29.3 taps a clock; list: per evaluated pixel and observation)
-TAP_INSTR = {"block": 4.4, "list": 7.5, "fp32": 10.0, "fp32_expanded": 6.0, "fp32_expanded_pairs": 3.5, "fp32_sparse": 15.0, "fp16_sparse": 18.5}
+TAP_INSTR = {"block": 4.4, "list": 7.5, "fp32": 10.0, "fp32_expanded": 6.0, "fp32_expanded_pairs": 3.5, "fp32_sparse": 15.0}
 ALU_PEAKS = os.path.join(ROOT, "profiles", "alu_peaks.json")
 STAGES = ((4, 5.0, 20.0), (2, 5.0, 20.0))
 L2_FLUSH_BYTES = 256 << 20
@@ -90,7 +90,76 @@ def parse():
                          "per-kernel table then comes from a separate untimed pass), 1 around every kernel")
     ap.add_argument("--serve-seconds", type=float, default=60.0,
                     help="duration of the paper-rate serving run (16 viewpoints x 30 fps)")
+    ap.add_argument("--details", default="",
+                    help="also write the full record (every tuner candidate, per-view error, per-kernel roofline "
+                         "and method note) to this file; the line on stdout is a summary of it")
     return ap.parse_args()
+
+
+# ---------------------------------------------------------------------------
+# the line on stdout
+# ---------------------------------------------------------------------------
+def _sig(x):
+    """Nested floats at six significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: _sig(v) for k, v in x.items()}
+    return [_sig(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def _filters(choice):
+    """The chosen kernel of each filter stage: kernel, loop, form, rows per thread, warps, tile."""
+    out = []
+    for s in choice["stages"]:
+        c = s["chosen"]
+        out.append(f"{c['kernel']}/{c.get('loop', 'gather')} {c['form']} kp{c['kp']} nw{c['warps']} "
+                   f"{c['tile'][0]}x{c['tile'][1]}" + (f" {c['tuned_us']:.1f} us" if "tuned_us" in c else ""))
+    return out
+
+
+def _pick(d, *keys):
+    return d and {k: d[k] for k in keys if k in d}
+
+
+def compact_line(out):
+    """The line for stdout: the headline's numbers as they are, what explains them in a few fields each.
+    (The full record is some 24 KB, more than what reads one line of a log may keep.)"""
+    head = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "clocks", "gpu_launches")
+    line = {k: out[k] for k in head}
+    line["config"] = out["config"]
+    line["latency_ms_per_step"] = out["latency_ms_per_step"]
+    r = out["roofline"]
+    line["roofline"] = dict(_pick(r, "kernel", "bound", "achieved", "peak", "unit", "frac", "traffic", "avg_launch_us",
+                                  "peak_basis"), peak_live=_pick(r.get("peak_live"), "taps_per_s", "binds"))
+    line["path_roofline"] = _pick(out["path_roofline"], "ideal_us_per_step", "measured_us_per_step", "frac")
+    line["kernels_us"] = {k: v["avg_us"] for k, v in out["kernels"].items()}
+    line["filter_kernels"] = _filters(out["filter_kernels"])
+    e = out["e2e"]
+    line["e2e"] = e and dict({k: v for k, v in e.items() if k != "host_link"},
+                             host_link=_pick(e["host_link"], "h2d_GBps", "d2h_GBps", "both_GBps", "bound_frames_per_s",
+                                             "duplex_frames_per_s"))
+    c = out["cpu_baseline"]
+    line["cpu_baseline"] = c and _pick(c, "value", "unit", "cores", "kind", "sample")
+    f = out["fp16"]
+    line["fp16"] = f and dict(_pick(f, "precision", "value", "unit", "ms_per_step", "jbf_stage2_avg_us"),
+                              filter_kernels=_filters(f["filter_kernels"]))
+    line["configs"] = out["configs"] and {
+        name: dict(_pick(w, "value", "ms_per_step", "gpu_launches"), path_frac=w["path_roofline"]["frac"],
+                   filter_kernels=_filters(w["filter_kernels"]),
+                   **({"cpu_fps": w["cpu_baseline"]["value"],
+                       "error_vs_oracle": _pick(w["cpu_baseline"]["error_vs_oracle"], "all_masks_exact",
+                                                "pixels_over_bar", "max_abs_m", "max_rel")}
+                      if "cpu_baseline" in w else {}))
+        for name, w in out["configs"].items()}
+    s = out["serving"]
+    line["serving"] = s and {
+        k: dict(_pick(v, "completed_frames", "frames_per_s", "e_again_retries", "buffer_waits"),
+                **{f"{q}_ms": v["latency_ms"][q] for q in ("p50", "p99", "max")}) if isinstance(v, dict) else v
+        for k, v in s.items() if k != "note"}
+    keep = {k: line[k] for k in head}
+    return dict(_sig(line), **keep)
 
 
 # ---------------------------------------------------------------------------
@@ -979,7 +1048,8 @@ def ours_arm(a, rank, world, local_rank):
         "gpu_launches": gpu_launches,
         "e2e": e2e,
         "cpu_baseline": cpu,
-        "fp16": fp16 and {"precision": "full-resolution stage: FP16 guide and weights, FP32 sums", **fp16},
+        "fp16": fp16 and {"precision": "FP16 context (guide and weights of the full-resolution stage may be FP16; "
+                                      "filter_kernels says what ran)", **fp16},
         "configs": configs or None,
         "serving": serving and {"viewpoints": "16 (1080p/720p/540p mixed, 1-3 sweeps each)",
                                 "paper_rate_seconds": a.serve_seconds,
@@ -988,7 +1058,10 @@ def ours_arm(a, rank, world, local_rank):
                                         "launched so far by the context and the most in flight at once",
                                 **serving},
     }
-    print(json.dumps(out), flush=True)
+    if a.details:
+        with open(a.details, "w") as f:
+            json.dump(out, f)
+    print(json.dumps(compact_line(out)), flush=True)
 
 
 def main():
