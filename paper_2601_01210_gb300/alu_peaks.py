@@ -50,12 +50,6 @@ FORMS = {
     # position): row offset, squared distance, 4 fma exponent, 2 sums, half the column terms of the
     # two pixels a lane owns; window test (max, compare); half of the position's loads and loop work
     "fp32_sparse": {"fma": 9.0, "fma2": 0.0, "ex2": 1.0, "other": 5.0},
-    # the sparse form with FP16 weights (per evaluated pixel and position, half of a lane's pair):
-    # FP32 row offset, window test, squared distance and its kp product, the sums (num, weight,
-    # squared-depth term); half of the pair's half2 differences, squares and exponent (7 half2
-    # instructions) and of its ex2.approx.f16x2; packing and widening, the position's loads and
-    # loop work
-    "fp16_sparse": {"fma": 9.0, "fma2": 0.0, "ex2": 0.0, "ex2_h2": 0.5, "hfma2": 3.5, "other": 5.5},
 }
 
 
