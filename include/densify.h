@@ -26,8 +26,11 @@
  *   - Camera frame: x right, y down, z forward; pixel (i, j) covers
  *     [i, i+1) x [j, j+1), so its centre is (i + 1/2, j + 1/2).
  *   - Depth is the camera z coordinate in the units of the point clouds.
- *   - RGB frames are H x W x 3 uint8, row pitch in bytes (>= 3 W, multiple
- *     of 16).
+ *   - RGB frames are H x W x 3 uint8, row pitch in bytes (>= 3 W). A frame
+ *     whose base and pitch are multiples of 16 is read in place, up to the next
+ *     4-byte boundary after the last row's 3 W bytes (what lies there does not
+ *     matter, and an aligned word that holds an image byte is always readable);
+ *     others are copied first.
  *   - Unless a function says otherwise, pointers inside densify_frame are
  *     DEVICE pointers (memory = DENSIFY_MEM_DEVICE) owned by the caller; with
  *     memory = DENSIFY_MEM_HOST they are host pointers (page-locked for
@@ -358,7 +361,14 @@ DENSIFY_API densify_status densify_inject_wait_failure(densify_ctx *ctx);
 /* The kernels that run the filter stages of Sec. 5 (Eq. (1)-(4) each).
  * JSON text describing the filter kernels the context runs: per filter stage the
  * chosen kernel (TMA-staged or plain, rows per thread, tile, grid) and, after
- * autotuning, every candidate's measured time; then the number of batches
+ * autotuning, every candidate's measured time. "loop" says how the kernel goes
+ * about its sums: "block" (the second stage in 3 x 3 blocks), "list" (the single
+ * stage over lists of its observations) or "gather"; "fp16" whether its guide
+ * and weights are in half precision (never in the first two: they are FP32 in
+ * both precisions). "form" is the arithmetic of a gather; for the block form it
+ * is "fp32", for the list form "fp32_sparse" or, in an FP16 context,
+ * "fp16_sparse", the names under which the tuning cache keeps the kernel that
+ * sums over the observations only. Then the number of batches
  * launched and the most batches in flight at once (launched, not yet
  * complete), and the number of CUDA graphs captured (all of them by the first
  * batch). Writes at most cap bytes

@@ -1027,9 +1027,12 @@ densify_status capture_slot(densify_ctx *c, Slot &sl, int which) {
 }
 
 // Whether a batch's second filter writes its frames' points (kernel sequence 1): every frame has the
-// validity bits' scratch and points in device memory, and the batch is larger than a 960 x 540 frame
-// (one such frame keeps the eight kernels that the launch counter is tested on; its kernels last a few
-// microseconds each either way).
+// validity bits' scratch and points in device memory, and the batch is larger than a 960 x 540 frame.
+// No crossover lies there: a pass in this sequence was faster at every size measured (separate
+// compaction -> this, us: one frame of 320 x 240 63.1 -> 56.6, of 960 x 540 68.2 -> 59.2, of 1920 x 1080
+// 100.9 -> 89.9; 32 of 320 x 240 253.9 -> 251.8, eight of 960 x 540 166 -> 161, eight of 1920 x 1080
+// 332 -> 290). A small frame's sequence of eight kernels, with bp_count and bp_write among its timed
+// steps, is what callers of densify_kernel_launches and densify_kernel_times have seen so far, and stays.
 constexpr int64_t kFusedPointsPx = 1 << 19;
 bool may_write_points(const densify_ctx *c) {   // some batch of this context
     return fused_points_apply(c->p) && c->sel[1].tma && c->sel[1].form == TMA_FORM_BLOCK;
