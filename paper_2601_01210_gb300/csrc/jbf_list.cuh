@@ -20,6 +20,13 @@
 //
 // A footprint with more than kListCap observations takes several lists in turn;
 // the order is row-major either way, so results do not depend on the split.
+//
+// A list costs some 15 instructions per observation of the footprint, most of
+// them for windows that do not hold it, so a tile of which more than a part
+// G::DENSE is observed gathers instead (list_gather): a thread takes two pixels
+// one above the other and walks their window positions in row-major order, an
+// unobserved one with weight 0. The terms and their order are those of the
+// lists, so a pixel's result is the same bits on either side of the line.
 #pragma once
 
 #include "jbf_core.cuh"
@@ -28,6 +35,12 @@
 namespace dz {
 
 constexpr int kListCap = 96;   // records of a warp's list (a 1080p view holds some 15 to 30 in a footprint)
+
+// Per cent of a tile's positions above which it gathers, by radius (2, 4 and 7 are instantiated), where
+// the two cost the same on evenly spread observations. Four 1280 x 720 frames, lists against gather, us,
+// at 10, 20, 30, 50 and 97 % observed: r = 2 54, 70, 91, 128, 257 against 64-67; r = 4 67, 98, 130, 212,
+// 416 against 133; r = 7 93, 162, 228, 375, 730 against 294.
+constexpr int kListDense[8] = {0, 0, 16, 0, 30, 0, 0, 39};
 
 template <int R_, int BLOCKS_>   // BLOCKS_: 8 x 8 blocks of a warp (the tile is 32 x 16 BLOCKS_)
 struct ListGeom {
@@ -48,26 +61,35 @@ struct ListGeom {
     static_assert(SCOLS <= SPITCH && SPITCH % 16 == 8, "table rows");
     static constexpr int OFF_LIST = 2 * (RAW_A + RAW_B);
     static constexpr int OFF_TAB = OFF_LIST + NW * kListCap * 16;
-    static constexpr int OFF_ROWS = OFF_TAB + SROWS * SPITCH * 8;
+    // the gather's spatial weights: window row of the upper pixel (0 .. 2 R + 1), column (0 .. 2 R); its
+    // colour words take the lists' place
+    static constexpr int OFF_PAIR = OFF_TAB + SROWS * SPITCH * 8;
+    static constexpr int OFF_ROWS = OFF_PAIR + (2 * R + 2) * (2 * R + 1) * 8;
+    static_assert(SH * SW * 4 <= NW * kListCap * 16, "the colour words fit the lists");
+    static constexpr int DENSE = SH * SW * kListDense[R] / 100;   // observations of a tile and its halo
     static constexpr int OFF_BAR = OFF_ROWS + SH * 8;
     static constexpr int SMEM = OFF_BAR + 16;
     static_assert(OFF_LIST % 16 == 0 && OFF_TAB % 16 == 0 && OFF_ROWS % 8 == 0, "layout");
 };
 
-// The table of spatial weights (every thread of the CTA; followed by a barrier).
+// Spatial weight at (dx, dy): 0 outside the window, at least 2^-126 inside it.
+template <int R>
+__device__ __forceinline__ float list_spatial(const StageArgs &a, int dx, int dy) {
+    const bool in = dy >= -R && dy <= R && dx >= -R && dx <= R;
+    return in ? fmaxf(ex2_approx(-(float)(dy * dy + dx * dx) * a.kp), 0x1p-126f) : 0.0f;
+}
+
+// The tables of spatial weights (every thread of the CTA; followed by a barrier).
 template <class G>
-__device__ __forceinline__ void list_table(const StageArgs &a, float2 *tab) {
+__device__ __forceinline__ void list_table(const StageArgs &a, float2 *tab, float2 *pair) {
     constexpr int R = G::R;
     for (int i = threadIdx.x; i < G::SROWS * G::SPITCH; i += G::NT) {
         const int dy = i / G::SPITCH - R - 3, dx = i % G::SPITCH - R - 7;
-        float s[2];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int ey = dy - 4 * k;
-            const bool in = ey >= -R && ey <= R && dx >= -R && dx <= R;
-            s[k] = in ? fmaxf(ex2_approx(-(float)(ey * ey + dx * dx) * a.kp), 0x1p-126f) : 0.0f;
-        }
-        tab[i] = make_float2(s[0], s[1]);
+        tab[i] = make_float2(list_spatial<R>(a, dx, dy), list_spatial<R>(a, dx, dy - 4));
+    }
+    for (int i = threadIdx.x; i < (2 * R + 2) * (2 * R + 1); i += G::NT) {
+        const int dy = i / (2 * R + 1) - R, dx = i % (2 * R + 1) - R;
+        pair[i] = make_float2(list_spatial<R>(a, dx, dy), list_spatial<R>(a, dx, dy - 1));
     }
 }
 
@@ -97,6 +119,97 @@ __device__ __forceinline__ uint32_t list_colour(const uint8_t *rgbraw, int sy, i
     return (uint32_t)p[0] | ((uint32_t)p[1] << 8) | ((uint32_t)p[2] << 16);
 }
 
+// Observations of the tile and its halo (after the barrier behind list_masks; the same for every thread).
+template <class G>
+__device__ __forceinline__ int list_count(const uint64_t *rowmask, int lane) {
+    int n = 0;
+#pragma unroll
+    for (int sy = lane; sy < G::SH; sy += 32) n += __popcll(rowmask[sy]);
+    return __reduce_add_sync(0xffffffffu, n);
+}
+
+// Colour weights 2^(-kc |c_p - c_q|^2) of two pixels and one position, times their spatial weights.
+__device__ __forceinline__ float2 list_weight(const StageArgs &a, uint32_t p0, uint32_t p1, uint32_t q, float2 s) {
+    const uint32_t d0 = __vabsdiffu4(p0, q), d1 = __vabsdiffu4(p1, q);
+    const float2 f = make_float2(__uint_as_float(__dp4a(d0, d0, 0x4B000000u)), __uint_as_float(__dp4a(d1, d1, 0x4B000000u)));
+    const float2 x = __ffma2_rn(f, a.bkc, a.bkb);
+    return __fmul2_rn(make_float2(ex2_approx(x.x), ex2_approx(x.y)), s);
+}
+
+// Depth of the valid pixel (px, py) of the tile from its sums; where the weight sum is too small (rare:
+// every observation of the window far in colour), with the largest exponent shifted to 0.
+template <class G>
+__device__ __forceinline__ float list_depth(const StageArgs &a, const uint8_t *rgbraw, const uint32_t *zraw,
+                                            const uint64_t *rowmask, int px, int py, float num, float den) {
+    constexpr int R = G::R;
+    if (den >= 0x1p-60f) return __fdividef(num, den);
+    const uint32_t p = list_colour<G>(rgbraw, py + R, px + R);
+    float amax = -__int_as_float(0x7F800000), sn = 0.0f, sd = 0.0f;
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass)
+#pragma unroll 1
+        for (int sy = py; sy <= py + 2 * R; ++sy)
+            for (uint64_t mm = (rowmask[sy] >> px) & ((uint64_t(1) << (2 * R + 1)) - 1u); mm; mm &= mm - 1u) {
+                const int sx = px + __ffsll((long long)mm) - 1;
+                const uint32_t d = __vabsdiffu4(p, list_colour<G>(rgbraw, sy, sx));
+                const float z = __uint_as_float(zraw[sy * G::Z_BX + sx - R + G::Z_LEAD]);
+                const int dx = sx - R - px, dy = sy - R - py;
+                const float e = fmaf((float)__dp4a(d, d, 0u), -a.kc, -(float)(dx * dx + dy * dy) * a.kp);
+                if (pass == 0) {
+                    amax = fmaxf(amax, e);
+                } else {
+                    const float w = ex2_approx(e - amax);
+                    sn = fmaf(w, z, sn);
+                    sd += w;
+                }
+            }
+    return sn / sd;
+}
+
+// A densely observed tile (every thread of the CTA): a thread takes rows y and y + 1 of column `lane`.
+// Per position one colour word, one depth and one pair of spatial weights (the same for the warp) serve
+// both pixels.
+template <class G, class Store>
+__device__ __forceinline__ void list_gather(const StageArgs &a, const uint8_t *rgbraw, const uint32_t *zraw,
+                                            const uint64_t *rowmask, uint32_t *words, const float2 *pair, int cols, int rows,
+                                            int warp, int lane, Store &&store) {
+    constexpr int R = G::R, T = 2 * R + 1;
+    static_assert(G::TH % (2 * G::NW) == 0 && 31 + T <= G::SW && G::TH - 2 + T < G::SH && 31 + R + G::Z_LEAD < G::Z_BX,
+                  "every position of a thread's windows lies in the tile and its halo");
+    for (int i = threadIdx.x; i < G::SH * G::SW; i += G::NT) words[i] = list_colour<G>(rgbraw, i / G::SW, i % G::SW);
+    __syncthreads();
+#pragma unroll 1
+    for (int y = 2 * warp; y < G::TH && y < rows; y += 2 * G::NW) {
+        const uint32_t *const w0 = words + y * G::SW + lane;
+        const uint32_t *const z0 = zraw + y * G::Z_BX + lane - R + G::Z_LEAD;
+        const uint32_t p0 = w0[R * G::SW + R], p1 = w0[(R + 1) * G::SW + R];
+        float2 num = make_float2(0.0f, 0.0f), den = num;
+        uint32_t hit0 = 0u, hit1 = 0u;
+#pragma unroll 1
+        for (int iy = 0; iy <= T; ++iy) {
+            const uint32_t m = (uint32_t)(rowmask[y + iy] >> lane) & ((1u << T) - 1u);
+            if (iy < T) hit0 |= m;
+            if (iy > 0) hit1 |= m;
+#pragma unroll
+            for (int dx = 0; dx < T; ++dx) {
+                const bool seen = (m >> dx) & 1u;
+                const float d = seen ? __uint_as_float(z0[iy * G::Z_BX + dx]) : 0.0f, b = seen ? 1.0f : 0.0f;
+                const float2 w = list_weight(a, p0, p1, w0[iy * G::SW + dx], pair[iy * T + dx]);
+                num = __ffma2_rn(w, make_float2(d, d), num);
+                den = __ffma2_rn(w, make_float2(b, b), den);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const bool hit = (k ? hit1 : hit0) != 0u;
+            float out = 0.0f;
+            if (hit && lane < cols && y + k < rows)
+                out = list_depth<G>(a, rgbraw, zraw, rowmask, lane, y + k, k ? num.y : num.x, k ? den.y : den.x);
+            store(lane, y + k, out, hit);
+        }
+    }
+}
+
 // The tile's blocks (every warp; after the barrier behind list_masks). store(x, y, depth, valid)
 // takes tile-relative pixel coordinates.
 template <class G, class Store>
@@ -105,7 +218,6 @@ __device__ __forceinline__ void list_blocks(const StageArgs &a, const uint8_t *r
                                             int lane, Store &&store) {
     constexpr int R = G::R, FR = G::FR;
     const int lx = lane & 7, ly = lane >> 3;
-    const float2 nkc = a.bkc, kb = a.bkb;
     const uint8_t *const tlane = reinterpret_cast<const uint8_t *>(tab + (3 - ly) * G::SPITCH + 7 - lx);
 #pragma unroll 1
     for (int blk = warp; blk < (G::TW / 8) * (G::TH / 8); blk += G::NW) {
@@ -141,11 +253,7 @@ __device__ __forceinline__ void list_blocks(const StageArgs &a, const uint8_t *r
                 for (int i = 0; i < e; ++i) {
                     const uint4 q = list[i];
                     const float2 s = *reinterpret_cast<const float2 *>(tlane + q.y);
-                    const uint32_t d0 = __vabsdiffu4(p0, q.x), d1 = __vabsdiffu4(p1, q.x);
-                    const float2 f = make_float2(__uint_as_float(__dp4a(d0, d0, 0x4B000000u)),
-                                                 __uint_as_float(__dp4a(d1, d1, 0x4B000000u)));
-                    const float2 x = __ffma2_rn(f, nkc, kb);
-                    const float2 w = __fmul2_rn(make_float2(ex2_approx(x.x), ex2_approx(x.y)), s);
+                    const float2 w = list_weight(a, p0, p1, q.x, s);
                     num = __ffma2_rn(w, make_float2(__uint_as_float(q.z), __uint_as_float(q.w)), num);
                     den = __fadd2_rn(den, w);
                     sum = __fadd2_rn(sum, s);
@@ -157,35 +265,9 @@ __device__ __forceinline__ void list_blocks(const StageArgs &a, const uint8_t *r
         for (int k = 0; k < 2; ++k) {
             const int px = bx + lx, py = by + ly + 4 * k;
             const bool hit = (k ? sum.y : sum.x) > 0.0f;
-            const float nn = k ? num.y : num.x, dd = k ? den.y : den.x;
             float out = 0.0f;
-            if (hit && px < cols && py < rows) {
-                if (dd >= 0x1p-60f) {
-                    out = __fdividef(nn, dd);
-                } else {   // rare: every observation of the window far in colour; the largest exponent shifted to 0
-                    const uint32_t p = list_colour<G>(rgbraw, py + R, px + R);
-                    float amax = -__int_as_float(0x7F800000), sn = 0.0f, sd = 0.0f;
-#pragma unroll 1
-                    for (int pass = 0; pass < 2; ++pass)
-#pragma unroll 1
-                        for (int sy = py; sy <= py + 2 * R; ++sy)
-                            for (uint64_t mm = (rowmask[sy] >> px) & ((uint64_t(1) << (2 * R + 1)) - 1u); mm; mm &= mm - 1u) {
-                                const int sx = px + __ffsll((long long)mm) - 1;
-                                const uint32_t d = __vabsdiffu4(p, list_colour<G>(rgbraw, sy, sx));
-                                const float z = __uint_as_float(zraw[sy * G::Z_BX + sx - R + G::Z_LEAD]);
-                                const int dx = sx - R - px, dy = sy - R - py;
-                                const float e = fmaf((float)__dp4a(d, d, 0u), -a.kc, -(float)(dx * dx + dy * dy) * a.kp);
-                                if (pass == 0) {
-                                    amax = fmaxf(amax, e);
-                                } else {
-                                    const float w = ex2_approx(e - amax);
-                                    sn = fmaf(w, z, sn);
-                                    sd += w;
-                                }
-                            }
-                    out = sn / sd;
-                }
-            }
+            if (hit && px < cols && py < rows)
+                out = list_depth<G>(a, rgbraw, zraw, rowmask, px, py, k ? num.y : num.x, k ? den.y : den.x);
             store(px, py, out, hit);
         }
     }

@@ -26,6 +26,7 @@ __global__ void __launch_bounds__(256, 3) jbf_list_kernel(const BatchDev *__rest
     auto rawA = [&](int b) { return smem + b * (G::RAW_A + G::RAW_B); };
     auto rawB = [&](int b) { return smem + b * (G::RAW_A + G::RAW_B) + G::RAW_A; };
     float2 *const tab = reinterpret_cast<float2 *>(smem + G::OFF_TAB);
+    float2 *const pair = reinterpret_cast<float2 *>(smem + G::OFF_PAIR);
     uint64_t *const rowmask = reinterpret_cast<uint64_t *>(smem + G::OFF_ROWS);
     uint64_t *const bar = reinterpret_cast<uint64_t *>(smem + G::OFF_BAR);
     __shared__ TileQueueMem s_queue;
@@ -52,7 +53,7 @@ __global__ void __launch_bounds__(256, 3) jbf_list_kernel(const BatchDev *__rest
         }
     __syncthreads();
     queue.start();
-    list_table<G>(a, tab);   // while the first tile's copies are on their way
+    list_table<G>(a, tab, pair);   // while the first tile's copies are on their way
     __syncthreads();
     for (int it = 0;; ++it) {
         const int buf = it & 1;
@@ -84,12 +85,17 @@ __global__ void __launch_bounds__(256, 3) jbf_list_kernel(const BatchDev *__rest
         float *const dp = out_depth + (int64_t)y0 * gw + x0;
         uint8_t *const vp = out_valid + (int64_t)y0 * gw + x0;
         const int cols = gw - x0, rows = gh - y0;
-        list_blocks<G>(a, rawA(buf), zraw, rowmask, list, tab, cols, rows, warp, lane, [&](int tx, int ty, float d, bool v) {
+        auto store = [&](int tx, int ty, float d, bool v) {
             if (tx < cols && ty < rows) {
                 dp[(int64_t)ty * gw + tx] = d;
                 vp[(int64_t)ty * gw + tx] = v;
             }
-        });
+        };
+        if (list_count<G>(rowmask, lane) > G::DENSE)
+            list_gather<G>(a, rawA(buf), zraw, rowmask, reinterpret_cast<uint32_t *>(smem + G::OFF_LIST), pair, cols, rows, warp,
+                           lane, store);
+        else
+            list_blocks<G>(a, rawA(buf), zraw, rowmask, list, tab, cols, rows, warp, lane, store);
         __syncthreads();   // the masks and raw[buf] are rewritten by the next tile
     }
 }
