@@ -191,6 +191,16 @@ extern "C" DENSIFY_API densify_status densify_frame_noalloc(const densify_params
         const int gw = kind == 1 ? Wc : W, gh = kind == 1 ? Hc : H;
         if (ker[i].tma) flag_words[i] = (size_t)cdiv(gw, ker[i].tile_w) * cdiv(gh, ker[i].tile_h);
     }
+    // A single stage of few taps, or over more points than pixels, stays in the plain kernel: the list form
+    // saves little there and its tile marks are one launch more. Pass times, list / plain, us: radius 2, one
+    // lidar sweep to three, 320 x 240 46-50 / 39-41, 1280 x 720 52-56 / 46-48, 1920 x 1080 58.4 / 59.8 at 0.004
+    // points a pixel, 68.2 / 68.2 at 0.09, 74.8 / 70.1 at 0.36; radius 4, 640 x 480 49.6 / 49.6 at 0.4,
+    // 51.6 / 45.5 at 1.2; radius 7, 64.0 / 64.5 at 1.2, 76.3 / 66.4 at 2.4.
+    int64_t points_in = 0;
+    for (int s = 0; s < f->num_scans; ++s) points_in += f->scans[s].count;
+    if (nst == 1 && ker[0].form == TMA_FORM_LIST &&
+        (points_in > npx || (ker[0].radius == 2 && (npx < (1 << 20) || 10 * points_in > npx))))
+        ker[0].tma = false;
     const size_t off_flags = o, off_bits = o + up256((flag_words[0] + flag_words[1]) * 4);
     const size_t bits_bytes = nst == 2 ? (size_t)cdiv(Wc, 32) * Hc * 4 : 0;
     const bool tma = (ker[0].tma || ker[1].tma) && !((uintptr_t)f->rgb & 15u) && !(f->rgb_pitch & 15) &&
