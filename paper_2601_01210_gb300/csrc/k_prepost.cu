@@ -22,7 +22,8 @@
 // store through a pointer read from the descriptor could alias it, which would
 // make the compiler read the descriptor again after every store). The motion mask
 // and its closing work on bit-packed rows, a warp per 32 x 32 tile; the occlusion
-// windows on 32 x 32 tiles staged in shared memory, for the observed pixels only;
+// windows on 32 x 32 tiles staged in shared memory, one pass along the rows and
+// one along the columns;
 // the contour test takes 4 consecutive pixels a thread.
 #include "desc.cuh"
 
@@ -253,15 +254,15 @@ __global__ void __launch_bounds__(kThreads) morph_kernel(const BatchDev *__restr
 
 // ---------------------------------------------------------------------------
 // Tiles of 32 x 32 output pixels; the tile and its rho halo are staged as z-buffer words, with one
-// 64-bit mask of observed columns per staged row. Only an observed pixel needs its window's mean, and
-// an empty cell adds nothing to a sum, so the observed pixels of the tile (a few percent) are gathered
-// into a list and each is summed by one thread over the observed cells of its window: FP32 row sums in
-// column order, added in row order, the same operations as over the whole window. What is left is the
-// copy of the z-buffer: every cell is written through, the removed ones then emptied.
-// Four 1080p three-scan frames, rho = 5: 57 -> 48 us (the sums of all windows, 22 additions a pixel and
-// as many for the counts); the copy's floor is 10. Bound: latency; a tile is four short phases between
-// barriers, the longest of them a warp or two of window sums (six blocks an SM overlap). Coordinates
-// divided by one thread a tile ahead, rows by shifts: 63 us before that.
+// 64-bit mask of observed columns per staged row. A tile with an observed pixel takes, for each of its 32
+// columns, every staged row's window sum and count (the cells in column order; an empty cell adds 0),
+// then for each observed pixel the sum of those over its window's rows, in row order: the FP32 sums of the
+// whole window in the fixed order. Every cell is written through, the removed ones then emptied.
+// Four 1280 x 720 frames, rho = 5: 25-26 us on lidar views of 0.1 to 3 points a pixel, 28 to 33 on evenly
+// spread depth of 2 to 100 % (rho = 2 22-27, rho = 12 45-65); the sums staged as floats and counts with
+// every window of a tile summed 31-33 (28-30, 68-70), one thread summing each observed pixel's own window
+// 27 at 0.1 points a pixel, 47 at 0.5, 92 at 3, and up to 388 on dense depth (rho = 12: 1757). Bound: latency,
+// three short phases between barriers (six blocks an SM overlap); the copy's floor is 4.
 constexpr int kMaxOccR = 16;
 struct OccFrame {
     const uint32_t *src;   // merged z-buffer
@@ -270,17 +271,19 @@ struct OccFrame {
     int32_t W, H, tiles_x;
 };
 
+// RHO > 0: the window radius fixed at compile time (the sums unrolled); 0: a.occ_radius.
+template <int RHO>
 __global__ void __launch_bounds__(kThreads, 6) occlusion_kernel(const BatchDev *__restrict__ B, const PrepostArgs a) {
     constexpr int T = kOccTile, S = T + 2 * kMaxOccR;   // staged rows and columns at most
     static_assert(T == 32 && S <= 64, "a row mask is one 64-bit word, a tile row one warp");
     __shared__ __align__(16) uint32_t sz[S * S];
     __shared__ uint64_t s_mask[S];
-    __shared__ uint16_t s_list[T * T];
-    __shared__ int s_n;
+    __shared__ float s_sum[S * T];     // row sums and counts of the windows of the tile's columns
+    __shared__ uint8_t s_cnt[S * T];
     __shared__ int s_at[2][3];   // frame, x0, y0 of this tile and the next (thread 0 divides for all)
     __shared__ int32_t s_pre[kMaxBatch + 1];
     __shared__ OccFrame s_f[kMaxBatch];
-    const int rho = a.occ_radius, rows = T + 2 * rho;
+    const int rho = RHO > 0 ? RHO : a.occ_radius, rows = T + 2 * rho;
     const int lead = (rho + 3) & ~3, cols = T + 2 * lead;   // at most 64 staged columns
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nf = B->n_frames;
@@ -336,39 +339,50 @@ __global__ void __launch_bounds__(kThreads, 6) occlusion_kernel(const BatchDev *
             if (lane == 0) s_mask[sy] = ml | ((uint64_t)mh << 32);
         }
         __syncthreads();
-        if (warp == 0) {   // the tile's observed pixels: lane r lists row r
-            const uint32_t own = (uint32_t)(s_mask[rho + lane] >> lead);
-            uint32_t at = __popc(own);
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t u = __shfl_up_sync(0xffffffffu, at, o);
-                if (lane >= o) at += u;
-            }
-            if (lane == 31) s_n = (int)at;
-            at -= __popc(own);
-            for (uint32_t m = own; m; m &= m - 1u) s_list[at++] = (uint16_t)(lane * T + __ffs(m) - 1);
-        }
-        __syncthreads();
-        const int n = s_n;
-        for (int i = threadIdx.x; i < n; i += kThreads) {
-            const int r = s_list[i] / T, c = s_list[i] % T, left = c + lead - rho;
+        // (the same in every warp) lane r: whether row r of the tile holds an observed pixel
+        if (__any_sync(0xffffffffu, (uint32_t)(s_mask[rho + lane] >> lead) != 0u)) {
             const uint64_t window = (uint64_t(2) << (2 * rho)) - 1u;
-            float sum = 0.0f;
-            int cnt = 0;
-            for (int dy = 0; dy <= 2 * rho; ++dy) {
-                uint64_t m = (s_mask[r + dy] >> left) & window;
-                if (!m) continue;   // an empty row adds 0
-                cnt += __popcll(m);
-                const float *const row = reinterpret_cast<const float *>(sz) + (r + dy) * S + left;
-                float s = 0.0f;
-                for (; m; m &= m - 1u) s = __fadd_rn(s, row[__ffsll((long long)m) - 1]);
-                sum = __fadd_rn(sum, s);
+            // row sums: 4 consecutive columns a thread, their windows' cells sliding through 4 registers
+            for (int i = threadIdx.x; i < rows * (T / 4); i += kThreads) {
+                const int r = i / (T / 4), x = 4 * (i % (T / 4)), left = x + lead - rho;
+                const uint32_t *const cell = sz + r * S + left;
+                auto depth = [&](int k) { return cell[k] != kEmpty ? __uint_as_float(cell[k]) : 0.0f; };
+                float v0 = depth(0), v1 = depth(1), v2 = depth(2), v3 = depth(3), s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
+#pragma unroll
+                for (int dx = 0; dx <= 2 * rho; ++dx) {
+                    s0 = __fadd_rn(s0, v0);
+                    s1 = __fadd_rn(s1, v1);
+                    s2 = __fadd_rn(s2, v2);
+                    s3 = __fadd_rn(s3, v3);
+                    v0 = v1;
+                    v1 = v2;
+                    v2 = v3;
+                    if (dx < 2 * rho) v3 = depth(dx + 4);
+                }
+                const uint64_t m = s_mask[r] >> left;
+                s_sum[r * T + x] = s0;
+                s_sum[r * T + x + 1] = s1;
+                s_sum[r * T + x + 2] = s2;
+                s_sum[r * T + x + 3] = s3;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) s_cnt[r * T + x + k] = (uint8_t)__popcll((m >> k) & window);
             }
-            const float z = __uint_as_float(sz[(r + rho) * S + c + lead]);
-            if (z > __fadd_rn(__fdiv_rn(sum, (float)cnt), a.occ_margin))
-                F.dst[(int64_t)(y0 + r) * F.zpitch + x0 + c] = kEmpty;   // after the barriers behind the copy
+            __syncthreads();
+            for (int r = warp; r < T; r += kThreads / 32) {
+                if (!(s_mask[r + rho] >> (lane + lead) & 1u)) continue;
+                float sum = 0.0f;
+                int cnt = 0;
+#pragma unroll
+                for (int dy = 0; dy <= 2 * rho; ++dy) {
+                    sum = __fadd_rn(sum, s_sum[(r + dy) * T + lane]);
+                    cnt += s_cnt[(r + dy) * T + lane];
+                }
+                const float z = __uint_as_float(sz[(r + rho) * S + lane + lead]);
+                if (z > __fadd_rn(__fdiv_rn(sum, (float)cnt), a.occ_margin))
+                    F.dst[(int64_t)(y0 + r) * F.zpitch + x0 + lane] = kEmpty;   // after the barriers behind the copy
+            }
         }
-        __syncthreads();   // the staged tile, masks and list are rewritten by the next tile
+        __syncthreads();   // the staged tile, masks and sums are rewritten by the next tile
     }
 }
 
@@ -515,7 +529,17 @@ cudaError_t launch_morph(const BatchDev *b, const PrepostArgs &a, bool dilate, i
 
 cudaError_t launch_occlusion(const BatchDev *b, const PrepostArgs &a, int grid, cudaStream_t s) {
     if (a.occ_radius < 1 || a.occ_radius > kMaxOccR) return cudaErrorInvalidValue;
-    occlusion_kernel<<<grid, kThreads, 0, s>>>(b, a);
+    switch (a.occ_radius) {
+    case 1: occlusion_kernel<1><<<grid, kThreads, 0, s>>>(b, a); break;
+    case 2: occlusion_kernel<2><<<grid, kThreads, 0, s>>>(b, a); break;
+    case 3: occlusion_kernel<3><<<grid, kThreads, 0, s>>>(b, a); break;
+    case 4: occlusion_kernel<4><<<grid, kThreads, 0, s>>>(b, a); break;
+    case 5: occlusion_kernel<5><<<grid, kThreads, 0, s>>>(b, a); break;
+    case 6: occlusion_kernel<6><<<grid, kThreads, 0, s>>>(b, a); break;
+    case 7: occlusion_kernel<7><<<grid, kThreads, 0, s>>>(b, a); break;
+    case 8: occlusion_kernel<8><<<grid, kThreads, 0, s>>>(b, a); break;
+    default: occlusion_kernel<0><<<grid, kThreads, 0, s>>>(b, a); break;
+    }
     return cudaGetLastError();
 }
 
@@ -528,7 +552,7 @@ int occupancy_prepost(KernelId k) {
     int n = 0;
     if (k == K_MOTION) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, motion_kernel, kThreads, 0);
     else if (k == K_DILATE || k == K_ERODE) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, morph_kernel, kThreads, 0);
-    else if (k == K_OCCLUSION) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, occlusion_kernel, kThreads, 0);
+    else if (k == K_OCCLUSION) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, occlusion_kernel<0>, kThreads, 0);
     else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, contour_kernel, kThreads, 0);
     return n > 0 ? n : 1;
 }
