@@ -1051,14 +1051,15 @@ bool batch_writes_points(const densify_ctx *c, const std::vector<uint64_t> &tk) 
 // The first batch captures, instantiates and uploads the graphs of both kernel sequences for every slot
 // (they are fixed once the filter kernels are chosen), so that no later batch pays for a capture, whatever
 // its size; without graphs it loads the second sequence's kernels. (Captured when a batch first took it,
-// the second sequence cost that batch 60 to 90 us in mid-traffic with two slots.)
-densify_status prepare_sequences(densify_ctx *c) {
+// the second sequence cost that batch 60 to 90 us in mid-traffic with two slots.) The batch's own sequence
+// comes first: captured second, its launches took 1 us longer on one 1080p frame and 2 on eight.
+densify_status prepare_sequences(densify_ctx *c, int first) {
     if (c->sequences_ready) return DENSIFY_OK;
     const int n = may_write_points(c) ? 2 : 1;
     if (c->p.use_graphs) {
-        for (int which = 0; which < n; ++which)
+        for (int k = 0; k < n; ++k)
             for (auto &sl : c->slots) {
-                densify_status st = capture_slot(c, sl, which);
+                densify_status st = capture_slot(c, sl, n == 1 ? 0 : k == 0 ? first : 1 - first);
                 if (st != DENSIFY_OK) return st;
             }
     } else if (n == 2) {
@@ -1129,7 +1130,7 @@ densify_status launch_batch(densify_ctx *c, int si) {
                              sl.stream),
            "rgb staging");
     }
-    if (densify_status st = prepare_sequences(c); st != DENSIFY_OK) return st;
+    if (densify_status st = prepare_sequences(c, which); st != DENSIFY_OK) return st;
     if (c->p.use_graphs) {
         CU(cudaGraphLaunch(sl.seq[which].exec, sl.stream), "graph launch");
     } else {
