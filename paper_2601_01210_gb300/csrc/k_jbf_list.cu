@@ -17,7 +17,7 @@ struct ListOut {
 // (the sparse form, whose loop walked row masks and tested windows: 205), r = 4 on 32 frames of
 // 320 x 240 38 us (the sparse form with half2 weights that FP16 contexts took: 82). Bound: issue, some
 // 15 instructions per observation and warp (two pixels a lane), of whose evaluations 225 of 484
-// (r = 7) fall inside their windows.
+// (r = 7) fall inside their windows; where tiles gather (the line: kListDense, jbf_list.cuh), issue too.
 template <int R, int BL>
 __global__ void __launch_bounds__(256, 3) jbf_list_kernel(const BatchDev *__restrict__ B, const StageArgs a) {
     using G = ListGeom<R, BL>;

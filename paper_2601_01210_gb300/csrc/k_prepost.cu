@@ -23,8 +23,7 @@
 // make the compiler read the descriptor again after every store). The motion mask
 // and its closing work on bit-packed rows, a warp per 32 x 32 tile; the occlusion
 // windows on 32 x 32 tiles staged in shared memory, one pass along the rows and
-// one along the columns;
-// the contour test takes 4 consecutive pixels a thread.
+// one along the columns; the contour test takes 4 consecutive pixels a thread.
 #include "desc.cuh"
 
 namespace dz {
@@ -261,8 +260,8 @@ __global__ void __launch_bounds__(kThreads) morph_kernel(const BatchDev *__restr
 // Four 1280 x 720 frames, rho = 5: 25-26 us on lidar views of 0.1 to 3 points a pixel, 28 to 33 on evenly
 // spread depth of 2 to 100 % (rho = 2 22-27, rho = 12 45-65); the sums staged as floats and counts with
 // every window of a tile summed 31-33 (28-30, 68-70), one thread summing each observed pixel's own window
-// 27 at 0.1 points a pixel, 47 at 0.5, 92 at 3, and up to 388 on dense depth (rho = 12: 1757). Bound: latency,
-// three short phases between barriers (six blocks an SM overlap); the copy's floor is 4.
+// 27 at 0.1 points a pixel, 47 at 0.5, 92 at 3, and up to 388 on dense depth (rho = 12: 1757). Bound: issue
+// (70 % of the slots on two 1080p frames), then the barriers between three short phases; the copy takes 4.
 constexpr int kMaxOccR = 16;
 struct OccFrame {
     const uint32_t *src;   // merged z-buffer

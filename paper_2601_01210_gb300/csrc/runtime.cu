@@ -328,8 +328,8 @@ std::vector<FilterSel> filter_candidates(const densify_params &p, int kind, int 
             const double kc = log2e / (2.0 * (double)st.sigma_c * (double)st.sigma_c);
             const double kp = log2e / (2.0 * (double)st.sigma_p * (double)st.sigma_p);
             if (p.kernel_variant == 0 && kc * 3.0 * 128.0 * 128.0 + kp * 2.0 * r * r <= kExpRange) {
-                // the single stage on the z-buffer (a few percent of the pixels observed): the sparse
-                // form first, whose work follows the observations; then the gather forms
+                // behind the list form: the sparse form, whose work follows the observations too, then the
+                // gather forms
                 if (kind == 0) add_tma(TMA_FORM_SPARSE);
                 add_tma(TMA_FORM_EXP_PAIRS);
                 add_tma(TMA_FORM_EXP);
